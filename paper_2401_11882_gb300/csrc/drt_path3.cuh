@@ -224,7 +224,7 @@ __device__ __forceinline__ void path3_geometry(const SmemTris& s, float3 tx, flo
 template <int MODE, int K>
 __device__ __forceinline__ bool path3_negligible(const Path3<K>& g, float gk, float floor) {
   if (g.degenerate || g.V == 0.f) return true;
-  return MODE == MODE_SIGMOID && g.V * gk < floor * (g.L * g.L);
+  return MODE == MODE_SIGMOID && g.V * fabsf(gk) < floor * (g.L * g.L);
 }
 
 // Power of one path of order K from its geometry (not degenerate): obstruction by every

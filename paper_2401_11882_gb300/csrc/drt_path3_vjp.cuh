@@ -531,7 +531,7 @@ struct VjpWalk3 {
     VjpPath3<K> R;
     vjp3_recompute<MODE, K>(s, tx, rx, cd, alpha, R);
     bool take = !R.degenerate && g != 0.f;
-    float V = gk;
+    float V = fabsf(gk);
 #pragma unroll
     for (int j = 1; j <= K; ++j) {
       take &= R.V[j] != 0.f;

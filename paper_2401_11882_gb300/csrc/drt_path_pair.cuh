@@ -272,8 +272,8 @@ __device__ __forceinline__ float2 path_power_pair(const SmemWalls& s, const Smem
     for (int j = 0; j <= K; ++j) vis_out[j] = f2(vis0[j], vis1[j]);
   }
   const float p0 = path_power_of<MODE, K>(g0, vis0, gk), p1 = path_power_of<MODE, K>(g1, vis1, gk);
-  const bool none0 = path_negligible<MODE, false>(g0, fabsf(gk), floor0);
-  const bool none1 = path_negligible<MODE, false>(g1, fabsf(gk), floor1);
+  const bool none0 = path_negligible<MODE, false>(g0, gk, floor0);
+  const bool none1 = path_negligible<MODE, false>(g1, gk, floor1);
   return f2(none0 || fabsf(p0) < floor0 ? 0.f : p0, none1 || fabsf(p1) < floor1 ? 0.f : p1);
 }
 
