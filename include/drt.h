@@ -565,7 +565,7 @@ drt_status drt_mlp_forward(const float* params, const void* shadow, const float*
 
 /* y[i] = MLP(x[i]) for any number n of rows in one launch and without workspace, each row
    as drt_mlp_forward computes it on the tcgen05 path; DRT_ERR_UNSUPPORTED while that path
-   is switched off. */
+   is switched off.  n = 0 launches nothing (x and y may then be NULL). */
 drt_status drt_mlp_predict(const float* params, const void* shadow, const float* freqs,
                            const float* x, int32_t n, float* y, void* stream);
 

@@ -808,10 +808,11 @@ drt_status drt_mlp_forward(const float* params, const void* shadow, const float*
 
 drt_status drt_mlp_predict(const float* params, const void* shadow, const float* freqs,
                            const float* x, int32_t n, float* y, void* stream) {
-  if (!params || !a16(shadow) || !freqs || !x || !y)
+  if (!params || !a16(shadow) || !freqs)
     return mlp_fail(DRT_ERR_INVALID_ARG, "NULL or misaligned pointer");
   if (n < 0) return mlp_fail(DRT_ERR_INVALID_ARG, "n < 0");
-  if (n == 0) return DRT_OK;
+  if (n == 0) return DRT_OK;   // no rows: x and y may be NULL
+  if (!x || !y) return mlp_fail(DRT_ERR_INVALID_ARG, "x or y is NULL");
   int* status = g_tc_mode.load() != 0 ? tc_status_ptr() : nullptr;
   if (!status) return mlp_fail(DRT_ERR_UNSUPPORTED, "drt_mlp_predict needs the tcgen05 path");
   const cudaError_t e = launch_fused_forward(params, static_cast<const mlp::bf16*>(shadow), freqs, x, n,
