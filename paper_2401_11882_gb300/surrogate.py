@@ -85,9 +85,14 @@ class SurrogateMLP:
     def forward(self, x: torch.Tensor) -> torch.Tensor:
         """Predictions for x [N, 2] (float32, any N): one launch over all rows, or chunks of
         the batch size where the tcgen05 path is switched off."""
-        x = x.to(self.device, torch.float32).contiguous()
+        x = x.to(self.device, torch.float32)
         N = x.shape[0]
         out = torch.empty(N, device=self.device)
+        if N and (x.dim() != 2 or x.shape[1] != 2):   # rows of two: a column goes to both
+            rows = torch.empty(N, 2, device=self.device)
+            rows[:] = x   # raises where x does not broadcast
+            x = rows
+        x = x.contiguous()
         if N <= _MAX_ROWS:
             status = _lib.load().drt_mlp_predict(
                 _ptr(self.params), _ptr(self.shadow), _ptr(self.freqs), _ptr(x), N, _ptr(out),
