@@ -415,7 +415,7 @@ __device__ __forceinline__ float3 shfl3(float3 v, int src) {
 template <int MODE>
 __device__ __forceinline__ float receiver_floor3(const SmemTris& s, int W, float3 tx, float3 rx,
                                                  float alpha, float gamma, long long n_cand) {
-  if (MODE != MODE_SIGMOID || !(gamma >= 0.f)) return 0.f;
+  if (MODE != MODE_SIGMOID || !has_floors(gamma, n_cand)) return 0.f;
   Cand cd;
   cd.k = 0;
 #pragma unroll
