@@ -106,7 +106,7 @@ __device__ __forceinline__ void sigmoid_visibility3(const SmemTris& s, int W, co
   for (int j = 0; j <= K; ++j) vn[j] = vd[j] = 1.f;
   for (int w0 = 0; w0 < W; w0 += 8) {
     const int w1 = min(w0 + 8, W);
-#pragma unroll 1
+#pragma unroll(K == 0 ? 2 : 1)   // K == 0: see WALL_TURN
     for (int w = w0; w < w1; ++w) {
       const float4 P = s.P[w], M0 = s.M0[w], M1 = s.M1[w], M2 = s.M2[w];
       bool cop[K + 2];   // w in the plane of reflection j's triangle

@@ -188,7 +188,7 @@ __device__ __forceinline__ void vjp3_factor_sweep(const SmemTris& s, int w0, int
     float others = 1.f, v = nz[j];
 #pragma unroll
     for (int i = 0; i <= K; ++i) others *= i == j ? 1.f : nz[i];
-#pragma unroll 1
+#pragma unroll(K == 0 ? 2 : 1)   // K == 0: see WALL_TURN
     for (int w = w0; w < w1; ++w) {
       if (((w - w0) & 7) == 0) {
         dead |= others * v < stop;

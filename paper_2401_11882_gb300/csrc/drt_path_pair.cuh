@@ -113,6 +113,11 @@ __device__ __forceinline__ void hard_visibility_pair(const SmemWalls& s, const S
       }
       if (__all_sync(0xffffffffu, z0 && z1)) break;
     }
+    if (K == 0 && w0 + 8 <= W) {   // see WALL_TURN
+#pragma unroll
+      for (int i = 0; i < 8; ++i) wall(w0 + i);
+      continue;
+    }
     const int we = min(w0 + 8, W);
 #pragma unroll HARD_UNROLL
     for (int w = w0; w < we; ++w) wall(w);
@@ -173,13 +178,14 @@ __device__ __forceinline__ void sigmoid_visibility_pair(const SmemWalls& s, cons
       vd[j] = mul2(vd[j], den);
     }
   };
+  constexpr bool WHOLE = UNROLL == SIG_UNROLL_ALL || K == 0;   // K == 0: see WALL_TURN
   for (int w0 = 0; w0 < W; w0 += 8) {
-    if (UNROLL == SIG_UNROLL_ALL && w0 + 8 <= W) {
+    if (WHOLE && w0 + 8 <= W) {
 #pragma unroll
       for (int i = 0; i < 8; ++i) wall(w0 + i);
     } else {
       const int we = min(w0 + 8, W);
-#pragma unroll(UNROLL == SIG_UNROLL_ALL ? 1 : UNROLL)
+#pragma unroll(WHOLE ? 1 : UNROLL)
       for (int w = w0; w < we; ++w) wall(w);
     }
 #pragma unroll
@@ -187,7 +193,7 @@ __device__ __forceinline__ void sigmoid_visibility_pair(const SmemWalls& s, cons
       vis[j] = mul2(vis[j], f2(__fdividef(vn[j].x, vd[j].x), __fdividef(vn[j].y, vd[j].y)));
       vn[j] = vd[j] = one;
     }
-    if (UNROLL != SIG_UNROLL_ALL) {
+    if (!WHOLE) {
       float2 all = vis[0];
 #pragma unroll
       for (int j = 1; j <= K; ++j) all = mul2(all, vis[j]);

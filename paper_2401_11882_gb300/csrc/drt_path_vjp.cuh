@@ -115,9 +115,14 @@ __device__ __forceinline__ void sigmoid_vis_sweep(const VSmem& s, int W, const C
     }
   };
   for (int w0 = 0; w0 < W; w0 += 8) {
-    const int we = min(w0 + 8, W);
+    if (K == 0 && w0 + 8 <= W) {   // see WALL_TURN
+#pragma unroll
+      for (int i = 0; i < 8; ++i) wall(w0 + i);
+    } else {
+      const int we = min(w0 + 8, W);
 #pragma unroll 1
-    for (int w = w0; w < we; ++w) wall(w);
+      for (int w = w0; w < we; ++w) wall(w);
+    }
 #pragma unroll
     for (int j = 0; j <= K; ++j) {
       nz[j] *= __fdividef(vn[j], vd[j]);
@@ -253,17 +258,21 @@ __device__ __forceinline__ void vjp_factor_sweep(const VSmem& s, int w0, int w1,
   for (int j = 0; j <= K; ++j) {
     float v = nz[j];
 #pragma unroll 1
-    for (int w = w0; w < w1; ++w) {
-      if (((w - w0) & 7) == 0 && __all_sync(FULL, dead)) return;
-      const float4 G = s.G[w];
-      const float4 E = s.E[w];
-      const float x1 = line_dist(G, P.Qx[j], P.Qy[j]), y1 = line_dist(G, P.Qx[j + 1], P.Qy[j + 1]);
-      const float x2 = fmaf(P.mx[j], E.x, fmaf(P.my[j], E.y, -P.mq[j]));
-      const float y2 = fmaf(P.mx[j], E.z, fmaf(P.my[j], E.w, -P.mq[j]));
-      const float f = leg_wall<MODE, false>(x1, y1, x2, y2, alpha).f;
-      if (!((j >= 1 && w == cd.w[j - 1]) || (j < K && w == cd.w[j]))) {
-        dead |= f == 0.f;
-        v *= f;
+    for (int wb = w0; wb < w1; wb += 8) {
+      if (__all_sync(FULL, dead)) return;
+      const int we = min(wb + 8, w1);
+#pragma unroll(WALL_TURN<K, 1>)
+      for (int w = wb; w < we; ++w) {
+        const float4 G = s.G[w];
+        const float4 E = s.E[w];
+        const float x1 = line_dist(G, P.Qx[j], P.Qy[j]), y1 = line_dist(G, P.Qx[j + 1], P.Qy[j + 1]);
+        const float x2 = fmaf(P.mx[j], E.x, fmaf(P.my[j], E.y, -P.mq[j]));
+        const float y2 = fmaf(P.mx[j], E.z, fmaf(P.my[j], E.w, -P.mq[j]));
+        const float f = leg_wall<MODE, false>(x1, y1, x2, y2, alpha).f;
+        if (!((j >= 1 && w == cd.w[j - 1]) || (j < K && w == cd.w[j]))) {
+          dead |= f == 0.f;
+          v *= f;
+        }
       }
     }
     nz[j] = v;
@@ -687,7 +696,7 @@ __device__ __forceinline__ void path_vjp(const VSmem& s, int W, float2 tx, float
     float Wa[K + 1];
 #pragma unroll
     for (int j = 0; j <= K; ++j) Wa[j] = (zc[j] == 0) ? visb[j] * nz[j] * alpha : 0.f;
-#pragma unroll 1
+#pragma unroll(K == 0 ? 2 : 1)
     for (int w = 0; w < W; ++w) {
       const float4 G = s.G[w];
       const float4 E = s.E[w];
@@ -761,7 +770,7 @@ __device__ __forceinline__ void path_vjp(const VSmem& s, int W, float2 tx, float
       if (!live_leg[j]) continue;
       const float q0x = Qx[j], q0y = Qy[j], q1x = Qx[j + 1], q1y = Qy[j + 1];
       float b0x = 0.f, b0y = 0.f, b1x = 0.f, b1y = 0.f, ax = 0.f, ay = 0.f, as = 0.f;
-#pragma unroll 1
+#pragma unroll(K == 0 ? 2 : 1)
       for (int w = 0; w < W; ++w) {
         const float4 G = s.G[w];
         const float4 E = s.E[w];
@@ -776,7 +785,9 @@ __device__ __forceinline__ void path_vjp(const VSmem& s, int W, float2 tx, float
         const float v0 = fb * lw.dx1, v1 = fb * lw.dy1;       // n . Q_j - c, n . Q_{j+1} - c
         const float x2b = fb * lw.dx2, y2b = fb * lw.dy2;     // m . (A - Q_j), m . (B - Q_j)
         const bool any = (v0 != 0.f) | (v1 != 0.f) | (x2b != 0.f) | (y2b != 0.f);
-        if (!__any_sync(FULL, any)) continue;   // most walls leave a leg alone
+        // most walls leave a leg alone (asking costs more than it saves where a line of
+        // sight has no wall adjoint to add)
+        if ((WG || K > 0) && !__any_sync(FULL, any)) continue;
         b0x = fmaf(v0, G.x, b0x);
         b0y = fmaf(v0, G.y, b0y);
         b1x = fmaf(v1, G.x, b1x);

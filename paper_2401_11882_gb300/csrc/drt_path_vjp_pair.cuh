@@ -142,7 +142,7 @@ __device__ __forceinline__ void sigmoid_vis_sweep_pair(const VSmem& s, const Sme
   };
   for (int w0 = 0; w0 < W; w0 += 8) {
     const int we = min(w0 + 8, W);
-#pragma unroll SIG_UNROLL
+#pragma unroll(WALL_TURN<K, SIG_UNROLL>)
     for (int w = w0; w < we; ++w) wall(w);
 #pragma unroll
     for (int j = 0; j <= K; ++j) {
