@@ -37,8 +37,12 @@ namespace {
 
 // SAVED: the sigmoid's leg visibilities come from a.saved (the forward's) instead
 // of the first wall sweep.
+// With the wall gradient two CTAs an SM are asked for: left to itself the compiler gave the
+// sigmoid with saved visibilities 149 registers, one CTA (128 walls x 1024 receivers,
+// K = 2, GB300: 25.0 ms, with two 16.8).
 template <int MODE, bool WG, bool SAVED = false>
-__global__ void __launch_bounds__(256, MODE == MODE_SIGMOID ? 0 : 2) vjp_kernel(const VjpArgs a) {
+__global__ void __launch_bounds__(256, MODE == MODE_SIGMOID && !WG ? 0 : 2)
+    vjp_kernel(const VjpArgs a) {
   extern __shared__ float4 smem[];
   __shared__ VjpQueue queues[MODE == MODE_SIGMOID ? 1 : 8];
   const float2 tx = make_float2(__ldg(a.tx), __ldg(a.tx + 1));
