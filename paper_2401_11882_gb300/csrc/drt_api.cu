@@ -145,8 +145,10 @@ drt_status decompose(const drt_scene* sc, const drt_tile* t, Kernel kern, Decomp
   // some 64 units (the resident warps take them as they go), within bounds.  The walks
   // queue their paths and a unit's last batch is partly empty, so large scenes want large
   // units: 8..256 for the power and field forwards, 32..512 for the dense adjoints (up to
-  // three stages of 32 or 64 paths), 32..128 for the sigmoid's, of which far more paths
-  // reach the last stage.  A scene with fewer units of the lower bound than the chip holds
+  // three stages of 32 or 64 paths).  Of the sigmoid's paths far more reach the last stage:
+  // 8..64 for its 2D forwards (a unit of 256 takes long enough to leave SMs idle at the end:
+  // 128 walls x 16384 receivers, K = 2, GB300, 256 / 128 / 64: 21.5 / 20.6 / 20.1 ms; the
+  // forward that saves every visibility 90.5 / 88.4 / 88.8), 32..128 for its adjoints.  A scene with fewer units of the lower bound than the chip holds
   // warps (16 an SM) is bound by the latency of one unit instead: it takes units down to
   // one candidate, until there is one for every warp.  The path finder queues nothing: 1..64.
   // Units of 64 candidates left small scenes on a few warps: finder, 17 walls x 400
@@ -162,7 +164,7 @@ drt_status decompose(const drt_scene* sc, const drt_tile* t, Kernel kern, Decomp
   long long least = 32, most = 512;
   if (forward) {
     least = 8;
-    most = 256;
+    most = kern != FWD3 && sc->smoothing == DRT_SMOOTH_SIGMOID ? 64 : 256;
   } else if (finder) {
     least = 1;
     most = 64;
