@@ -613,10 +613,11 @@ drt_status drt_mlp_adam(float* params, float* m, float* v, const float* grad, in
    DRT_NOALLOC_SCRATCH_BYTES compiled into the library's device image, which
    every GPU that loads the library keeps until the process exits, and calls no
    allocator.  Same arguments as drt_forward with default tiling (scene: host
-   pointer; power: [n_rx] device, overwritten); the result equals drt_forward's
-   within FP32 rounding: for large n_rx the candidate chunk is larger than the
-   default one, so the per-chunk partial sums are grouped differently.  Two
-   calls with the same arguments give the same bits.
+   pointer; power: [n_rx] device, overwritten); the result equals drt_forward's,
+   bit for bit where that call's workspace fits the array, within FP32 rounding
+   otherwise (the candidate chunk is then larger than the default one, so the
+   per-chunk partial sums are grouped differently).  Two calls with the same
+   arguments give the same bits.
    - Limit: one partial sum per (candidate chunk, receiver) must fit, so
      n_rx <= DRT_NOALLOC_SCRATCH_BYTES / 4; above DRT_MAX_WALLS walls the
      staged wall records (128 bytes per wall) share the array and lower that

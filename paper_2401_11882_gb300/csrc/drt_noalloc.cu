@@ -86,6 +86,13 @@ extern "C" drt_status drt_forward_noalloc(const drt_scene* scene, float* power, 
   drt_status st = drt_forward_workspace_size(scene, nullptr, &default_need);
   if (st != DRT_OK) return st;
   if (scene->n_rx == 0) return drt_forward(scene, nullptr, power, nullptr, 0, stream);
+  // The default units where their partial sums (and staged wall records) fit, as drt_forward
+  // takes them; otherwise as many chunks as fit.
+  if (default_need <= DRT_NOALLOC_SCRATCH_BYTES) {
+    void* scratch = nullptr;
+    if ((st = scratch_on_current_device(&scratch)) != DRT_OK) return st;
+    return drt_forward(scene, nullptr, power, scratch, DRT_NOALLOC_SCRATCH_BYTES, stream);
+  }
   // One partial sum per (candidate chunk, receiver): choose the chunk so that they
   // fit beside the staged wall records of a scene with more walls than shared
   // memory holds (at most 8 float4 per wall, after the partial sums rounded up to 16
