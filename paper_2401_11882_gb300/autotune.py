@@ -3,26 +3,31 @@
 Times a set of candidate tile shapes (warps per CTA, candidates per work
 unit, resident CTAs per SM, one or two receivers per lane) with CUDA events on
 the current stream (inside the library: drt_tune_forward) and keeps the
-fastest.  Results are cached on disk, keyed by GPU name, smoothing, order
-K and the power-of-two buckets of the wall and receiver counts; a later call
-with a key in the cache costs no timing.  Cache file: $DRT_TUNE_CACHE, else
+fastest.  Results are cached on disk, keyed by the kernels' sources, GPU name,
+smoothing, order K and the power-of-two buckets of the wall and receiver counts;
+a later call with a key in the cache costs no timing.  Cache file: $DRT_TUNE_CACHE, else
 ~/.cache/drt_gb300/tune.json.
 """
 from __future__ import annotations
 
+import functools
+import hashlib
 import json
 import math
 import os
 import threading
 from dataclasses import asdict, replace
 
+from . import _build
 from .ops import TileConfig
 
 _lock = threading.Lock()
 
+# cands_per_unit 0 is the library's own rule (1 to 256 by scene size); the first candidate is
+# its default tile, which therefore wins a tie
 FORWARD_CANDIDATES = [
     TileConfig(warps_per_cta=w, cands_per_unit=c, ctas_per_sm=o)
-    for w in (4, 8) for c in (16, 32, 64, 128) for o in (0, 2)
+    for w in (8, 4) for c in (0, 16, 32, 64, 128) for o in (0, 2)
 ]
 
 BATCH_CANDIDATES = [TileConfig(warps_per_cta=w, ctas_per_sm=o) for w in (4, 8) for o in (0, 1, 2)]
@@ -37,8 +42,18 @@ def _bucket(n: int) -> int:
     return 1 << max(0, math.ceil(math.log2(max(1, n))))
 
 
+@functools.lru_cache(maxsize=None)
+def kernels() -> str:
+    """A short digest of the library's sources: times of other kernels are not comparable."""
+    h = hashlib.sha256()
+    for path in sorted(_build._inputs()):
+        with open(path, "rb") as f:
+            h.update(os.path.basename(path).encode() + b"\0" + f.read() + b"\0")
+    return h.hexdigest()[:12]
+
+
 def forward_key(gpu: str, smoothing: str, max_order: int, n_walls: int, n_rx: int) -> str:
-    return f"fwd|{gpu}|{smoothing}|K{max_order}|W{_bucket(n_walls)}|R{_bucket(n_rx)}"
+    return f"fwd|{kernels()}|{gpu}|{smoothing}|K{max_order}|W{_bucket(n_walls)}|R{_bucket(n_rx)}"
 
 
 def load_cache(path: str | None = None) -> dict:
