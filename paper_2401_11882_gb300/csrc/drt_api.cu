@@ -127,7 +127,7 @@ constexpr long long MAX_PARTIALS = 1LL << 26;
 // (8 or 12 bytes); more tiles than this make one unit per tile.
 constexpr long long MAX_VJP_UNITS = 1LL << 22;
 
-// VJP_RX: the min-loss adjoint's one-receiver kernel (lanes = candidates)
+// VJP_RX: the min-loss adjoint's one-receiver kernel (one path per warp, lanes = walls)
 // VJP_TX: drt_vjp without the wall gradient (one receiver per lane)
 // VJP3_TX: drt3_vjp without the triangle gradient
 enum Kernel { FWD, VJP, VJP_TX, VJP_RX, FIELD, FIELD_VJP, FWD3, VJP3, VJP3_TX, FWD_MPT, FWD_FPT };
@@ -1063,10 +1063,7 @@ drt_status drt_min_loss_vjp(const drt_scene* scene, const drt_tile* tile, const 
   a.alpha = scene->alpha;
   gamma_powers(scene->refl_coef, a.gk);
   a.n_cand = d.n_cand;
-  a.chunk = 32;
-  a.n_chunks = (d.n_cand + 31) / 32;
   a.n_tiles = 1;
-  a.n_units = a.n_chunks;
   a.grad_power = nullptr;
   a.rx_index = argmin;
   a.grad_loss = grad_loss;
@@ -1080,7 +1077,7 @@ drt_status drt_min_loss_vjp(const drt_scene* scene, const drt_tile* tile, const 
   const long long warps = d.threads / 32;
   const long long most = std::max(1LL, std::min((long long)d.ctas, (long long)drx.ctas));
   a.chunk = (int)std::min(32LL, std::max(1LL, (d.n_cand + most * warps - 1) / (most * warps)));
-  a.n_units = (d.n_cand + a.chunk - 1) / a.chunk;
+  a.n_chunks = a.n_units = (d.n_cand + a.chunk - 1) / a.chunk;
   const int ctas = (int)std::min(most, (a.n_units + warps - 1) / warps);
   cudaError_t e = launch_vjp(a, scene->smoothing, ctas, d.threads,
                              static_cast<cudaStream_t>(stream));

@@ -184,7 +184,7 @@ __device__ __forceinline__ void vjp3_factor_sweep(const SmemTris& s, int w0, int
                                                   float* nz, bool& dead) {
 #pragma unroll
   for (int j = 0; j <= K; ++j) {   // one loop per leg, as vjp_factor_sweep
-    const float4 Pa = s.P[cd.w[j >= 1 ? j - 1 : 0]], Pb = s.P[cd.w[j < K ? j : 0]];
+    const float4 Pa = s.P[j >= 1 ? cd.w[j >= 1 ? j - 1 : 0] : 0], Pb = s.P[j < K ? cd.w[j < K ? j : 0] : 0];
     float others = 1.f, v = nz[j];
 #pragma unroll
     for (int i = 0; i <= K; ++i) others *= i == j ? 1.f : nz[i];
@@ -272,7 +272,7 @@ __device__ __forceinline__ void path_vjp3(const SmemTris& s, int W, float3 tx, f
   // delta_k = (1 - t) e0_k + t e1_k with e_k = m_k . Q - o_k)
 #pragma unroll
   for (int j = 0; j <= K; ++j) {   // one loop per leg, as vjp_factor_sweep
-    const float4 Pa = s.P[cd.w[j >= 1 ? j - 1 : 0]], Pb = s.P[cd.w[j < K ? j : 0]];
+    const float4 Pa = s.P[j >= 1 ? cd.w[j >= 1 ? j - 1 : 0] : 0], Pb = s.P[j < K ? cd.w[j < K ? j : 0] : 0];
     const float3 q0 = Q[j], q1 = Q[j + 1];
     float3 b0 = make_float3(0.f, 0.f, 0.f), b1 = b0;
 #pragma unroll 1

@@ -70,19 +70,17 @@ __device__ __forceinline__ void add_wall_adjoint(const VSmem& s, int w, float nb
 // product form (e = 2^-|z|, numerator and denominator products folded every 8
 // walls), the leg's own walls masked.  A factor that is exactly 0 (an FP32
 // underflow) makes the visibility 0, and so does a product that underflows; either
-// way the path's gradient is exactly 0 (see path_vjp), so no zero count is kept
-// (zc stays 0).  mxk, myk, mck: the leg's line scaled by alpha log2(e), as the
-// forward's.
+// way the path's gradient is exactly 0 (see path_vjp).  mxk, myk, mck: the leg's line
+// scaled by alpha log2(e), as the forward's.
 template <int K>
 __device__ __forceinline__ void sigmoid_vis_sweep(const VSmem& s, int W, const Cand& cd,
                                                   const float* Qx, const float* Qy,
                                                   const float* mxk, const float* myk,
-                                                  const float* mck, float* nz, int* zc) {
+                                                  const float* mck, float* nz) {
   float vn[K + 1], vd[K + 1];
 #pragma unroll
   for (int j = 0; j <= K; ++j) {
     nz[j] = vn[j] = vd[j] = 1.f;
-    zc[j] = 0;
   }
   // one wall's factors for every leg (the leg's own walls masked)
   auto wall = [&](int w) {
@@ -291,14 +289,14 @@ struct VjpFactorAdj {
 template <int K, bool FIELD>
 __device__ __forceinline__ void vjp_factor_adjoints(const VSmem& s, const Cand& cd,
                                                     const VjpPath<K>& P, const float* nz,
-                                                    const int* zc, float g, float gk,
+                                                    float g, float gk,
                                                     const FieldW* fw, VjpFactorAdj<K>& A) {
   constexpr int NF = 2 * K + 1;
   float F[NF];
 #pragma unroll
   for (int j = 1; j <= K; ++j) F[j - 1] = P.V[j];
 #pragma unroll
-  for (int j = 0; j <= K; ++j) F[K + j] = zc[j] ? 0.f : nz[j];
+  for (int j = 0; j <= K; ++j) F[K + j] = nz[j];
   float pre[NF + 1], suf[NF + 1];
   pre[0] = 1.f;
 #pragma unroll
@@ -622,14 +620,12 @@ __device__ __forceinline__ void path_vjp(const VSmem& s, int W, float2 tx, float
     dead |= all < least;
   }
   if (__all_sync(FULL, dead)) return;
-  // sweep 1: visibility as (product of non-zero factors, number of zero factors)
+  // sweep 1: each leg's visibility (a path with a factor of exactly 0 is dead)
   float nz[K + 1];
-  int zc[K + 1];
   float mxk[K + 1], myk[K + 1], mck[K + 1];   // sigmoid: the leg lines scaled by alpha log2(e)
 #pragma unroll
   for (int j = 0; j <= K; ++j) {
     nz[j] = 1.f;
-    zc[j] = 0;
     const float kap = alpha * LOG2E;
     mxk[j] = mx[j] * kap;
     myk[j] = my[j] * kap;
@@ -650,7 +646,7 @@ __device__ __forceinline__ void path_vjp(const VSmem& s, int W, float2 tx, float
 #pragma unroll
       for (int j = 0; j <= K; ++j) nz[j] = dead ? 1.f : nz[j];
     } else {
-      sigmoid_vis_sweep<K>(s, W, cd, Qx, Qy, mxk, myk, mck, nz, zc);
+      sigmoid_vis_sweep<K>(s, W, cd, Qx, Qy, mxk, myk, mck, nz);
     }
   } else if (vis) {
 #pragma unroll
@@ -669,7 +665,7 @@ __device__ __forceinline__ void path_vjp(const VSmem& s, int W, float2 tx, float
   if (dead) g = 0.f;
   // ------------------------------------------------ factor adjoints
   VjpFactorAdj<K> A;
-  vjp_factor_adjoints<K, FIELD>(s, cd, P, nz, zc, g, gk, fw, A);
+  vjp_factor_adjoints<K, FIELD>(s, cd, P, nz, g, gk, fw, A);
   const float* visb = A.visb;
 
   // ------------------------------------------------ sweep 2: obstruction adjoint
@@ -695,7 +691,7 @@ __device__ __forceinline__ void path_vjp(const VSmem& s, int W, float2 tx, float
     // reciprocal finite.
     float Wa[K + 1];
 #pragma unroll
-    for (int j = 0; j <= K; ++j) Wa[j] = (zc[j] == 0) ? visb[j] * nz[j] * alpha : 0.f;
+    for (int j = 0; j <= K; ++j) Wa[j] = visb[j] * nz[j] * alpha;
 #pragma unroll(K == 0 ? 2 : 1)
     for (int w = 0; w < W; ++w) {
       const float4 G = s.G[w];

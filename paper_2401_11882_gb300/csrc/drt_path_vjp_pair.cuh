@@ -284,16 +284,14 @@ __device__ __forceinline__ void path_vjp_pair(const VSmem& s, const SmemPairsVjp
     }
     // ---------------------------------------------- factor adjoints (per path)
     float nz0[K + 1], nz1[K + 1];
-    int zc[K + 1];
 #pragma unroll
     for (int j = 0; j <= K; ++j) {
       nz0[j] = vis[j].x;
       nz1[j] = vis[j].y;
-      zc[j] = 0;
     }
     VjpFactorAdj<K> A0, A1;
-    vjp_factor_adjoints<K, false>(s, cd0, P0, nz0, zc, g0, gk, nullptr, A0);
-    vjp_factor_adjoints<K, false>(s, cd1, P1, nz1, zc, g1, gk, nullptr, A1);
+    vjp_factor_adjoints<K, false>(s, cd0, P0, nz0, g0, gk, nullptr, A0);
+    vjp_factor_adjoints<K, false>(s, cd1, P1, nz1, g1, gk, nullptr, A1);
 #pragma unroll
     for (int j = 0; j <= K; ++j) {
       Wa[j] = f2(A0.visb[j] * nz0[j] * alpha, A1.visb[j] * nz1[j] * alpha);

@@ -242,12 +242,8 @@ def batch_tile_study(n_scenes=4096, tune_scenes=64, timed_steps=1, seed=0, devic
                      smoothing="hard_sigmoid") -> dict:
     """The batch autotuner on the 4096-scene batch: autotune.tune_batch times every
     candidate tile (warps per CTA x CTAs per SM) on the first tune_scenes scenes; the
-    full batch is then timed with the library's default tile, with the tuned tile, and
-    with the tuned tile and the flags DRT_TILE_CULL_INVALID and DRT_TILE_EXIT_BLOCKED,
-    which are accepted and change nothing (every walk leaves out the paths of validity
-    exactly 0 and the wall loop of blocked warps): the same losses bit for bit, in the
-    same time."""
-    from dataclasses import asdict, replace
+    full batch is then timed with the library's default tile and with the tuned tile."""
+    from dataclasses import asdict
     from . import autotune, workload
     full = scenes.scene_batch(n_scenes, seed, smoothing=smoothing)
     dev = torch.device(device)
@@ -266,16 +262,6 @@ def batch_tile_study(n_scenes=4096, tune_scenes=64, timed_steps=1, seed=0, devic
            "best": asdict(best)}
     out["default_tile"] = _time_full_batch(full, timed_steps, fl, evals, dev)
     out["tuned_tile"] = _time_full_batch(full, timed_steps, fl, evals, dev, tile=best)
-    skip = _time_full_batch(full, timed_steps, fl, evals, dev,
-                            tile=replace(best, cull_invalid=True))
-    skip.pop("tflops_by_convention")
-    out["tuned_tile_exact_skip"] = skip
-    for key, t in (("tuned_tile_blocked_exit", replace(best, exit_blocked=True)),
-                   ("tuned_tile_exact_skip_blocked_exit",
-                    replace(best, cull_invalid=True, exit_blocked=True))):
-        r = _time_full_batch(full, timed_steps, fl, evals, dev, tile=t)
-        r.pop("tflops_by_convention")
-        out[key] = r
     return out
 
 

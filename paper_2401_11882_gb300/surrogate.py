@@ -165,12 +165,14 @@ def sample_objective(scene, tx: np.ndarray, device="cuda", cull: bool = True,
 
     F does not depend on the order of the receivers, so they are passed in
     Z-order: the receivers of one warp are then near each other, and more
-    candidates are dropped for the whole warp at once.  One warp per CTA: a work unit (one sample, 64
-    receivers) is then never split between warps that wait for each other."""
+    candidates are dropped for the whole warp at once.  One warp per CTA: a work
+    unit (one sample, 64 receivers) is then never split between warps that wait for
+    each other.  ``cull`` is accepted without effect: paths of power exactly 0 are
+    always left out."""
     from . import scenes
     from .batched import BatchedDescent
     out = np.empty(tx.shape[0], np.float32)
-    tile = TileConfig(warps_per_cta=1, cull_invalid=cull and scene.smoothing != "sigmoid")
+    tile = TileConfig(warps_per_cta=1)
     rx = np.ascontiguousarray(scene.rx[scenes.spatial_order(scene.rx)])
     for s in range(0, tx.shape[0], chunk):
         part = np.asarray(tx[s:s + chunk], np.float32)
