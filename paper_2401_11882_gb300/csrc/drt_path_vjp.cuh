@@ -255,22 +255,30 @@ __device__ __forceinline__ void vjp_factor_sweep(const VSmem& s, int w0, int w1,
 #pragma unroll
   for (int j = 0; j <= K; ++j) {
     float v = nz[j];
-#pragma unroll 1
-    for (int wb = w0; wb < w1; wb += 8) {
-      if (__all_sync(FULL, dead)) return;
-      const int we = min(wb + 8, w1);
+    auto wall = [&](int w) {
+      const float4 G = s.G[w];
+      const float4 E = s.E[w];
+      const float x1 = line_dist(G, P.Qx[j], P.Qy[j]), y1 = line_dist(G, P.Qx[j + 1], P.Qy[j + 1]);
+      const float x2 = fmaf(P.mx[j], E.x, fmaf(P.my[j], E.y, -P.mq[j]));
+      const float y2 = fmaf(P.mx[j], E.z, fmaf(P.my[j], E.w, -P.mq[j]));
+      const float f = leg_wall<MODE, false>(x1, y1, x2, y2, alpha).f;
+      if (!((j >= 1 && w == cd.w[j - 1]) || (j < K && w == cd.w[j]))) {
+        dead |= f == 0.f;
+        v *= f;
+      }
+    };
+    if constexpr (K == 0) {   // see WALL_TURN
+      for (int wb = w0; wb < w1; wb += 8) {
+        if (__all_sync(FULL, dead)) return;
+        const int we = min(wb + 8, w1);
 #pragma unroll(WALL_TURN<K, 1>)
-      for (int w = wb; w < we; ++w) {
-        const float4 G = s.G[w];
-        const float4 E = s.E[w];
-        const float x1 = line_dist(G, P.Qx[j], P.Qy[j]), y1 = line_dist(G, P.Qx[j + 1], P.Qy[j + 1]);
-        const float x2 = fmaf(P.mx[j], E.x, fmaf(P.my[j], E.y, -P.mq[j]));
-        const float y2 = fmaf(P.mx[j], E.z, fmaf(P.my[j], E.w, -P.mq[j]));
-        const float f = leg_wall<MODE, false>(x1, y1, x2, y2, alpha).f;
-        if (!((j >= 1 && w == cd.w[j - 1]) || (j < K && w == cd.w[j]))) {
-          dead |= f == 0.f;
-          v *= f;
-        }
+        for (int w = wb; w < we; ++w) wall(w);
+      }
+    } else {
+#pragma unroll 1
+      for (int w = w0; w < w1; ++w) {
+        if (((w - w0) & 7) == 0 && __all_sync(FULL, dead)) return;
+        wall(w);
       }
     }
     nz[j] = v;
