@@ -142,7 +142,7 @@ __device__ __forceinline__ void path_field_pair(const SmemWalls& s, const SmemPa
 // SAVE: the visibilities of the paths that count for the adjoint are kept too.
 template <int MODE, bool SAVE>
 struct FieldEval {
-  static constexpr bool FLOORS = MODE == MODE_SIGMOID;
+  static constexpr bool FLOORS = MODE == MODE_SIGMOID, SAVES = SAVE;
   static constexpr float FLOOR = SAVE ? FLOOR_VJP : 1.f;
   const SmemWalls& s;
   const SmemPairs& p;
@@ -150,13 +150,13 @@ struct FieldEval {
   float2 tx;
   const float* ck;
   SavedVis saved;
-  template <int K>
+  template <int K, int UNROLL = SIG_UNROLL>
   __device__ __forceinline__ void operator()(const QueuedPath& q0, const QueuedPath& q1, float2& v0,
                                              float2& v1) const {
     // the sum takes what the plain field's takes; SAVE keeps the visibilities further down
     float2 vis[K + 1];
     bool keep0 = false, keep1 = false;
-    path_field_pair<MODE, K, SAVE>(s, p, a, tx, q0.rx, q0.cd, q0.floor, q1.rx, q1.cd, q1.floor, v0,
+    path_field_pair<MODE, K, SAVE, UNROLL>(s, p, a, tx, q0.rx, q0.cd, q0.floor, q1.rx, q1.cd, q1.floor, v0,
                                    v1, SAVE ? vis : nullptr, &keep0, &keep1);
     if (SAVE) {
       float va[K + 1], vb[K + 1];

@@ -1,4 +1,4 @@
-"""The hard sigmoid's dense adjoint at a small alpha, where every path counts and every wall has an
+"""Small alphas, where every path counts.  The hard sigmoid's dense adjoint, whose walls all have an
 adjoint from every leg: against the oracle, at walls around the sweeps' blocks of 8 and their split at
 a quarter of the walls, and around one tile of receivers; and its time."""
 import numpy as np
@@ -70,3 +70,27 @@ def test_the_adjoint_of_every_path_takes_under_twelve_forwards():
     s = (2, 1.0, "hard_sigmoid")
     forward = microseconds(lambda: ops.forward(w, t, r, *s))
     assert microseconds(lambda: ops.vjp(w, t, r, *s, g)) < 12 * forward
+
+
+@pytest.mark.parametrize("W,nx,ny,K,alpha", [(1, 1, 1, 1, 1.0), (7, 9, 7, 2, 1.0), (8, 8, 8, 2, 10.0), (9, 5, 13, 3, 10.0),
+                                             (17, 26, 25, 2, 30.0), (12, 64, 40, 2, 100.0), (6, 11, 6, 2, 0.0)])
+def test_sigmoid_paths_evaluated_without_stages_have_the_same_powers(oracle_mod, W, nx, ny, K, alpha):
+    """Tiles near the transmitter for their alpha evaluate every path, the others queue the ones that
+    count; the forward that saves visibilities always queues.  Same bits, also where a scene has tiles
+    of both kinds (alpha 30 and 100), and the oracle's powers."""
+    from parity import assert_power_close
+    from paper_2401_11882_gb300 import ops
+    rng = np.random.default_rng([W, nx])
+    gx, gy = np.meshgrid(np.linspace(0.03, 0.97, nx), np.linspace(0.05, 0.93, ny))
+    walls, tx, rx = (np.asarray(a, np.float32) for a in (
+        scenes.random_segments(rng, W), [0.41, 0.52], np.stack([gx.ravel(), gy.ravel()], 1)))
+    w, t, r = cuda(walls, tx, rx)
+    s = (K, alpha, "sigmoid")
+    for tile in (dict(), dict(cands_per_unit=7)):
+        P = ops.forward(w, t, r, *s, tile=ops.TileConfig(**tile))
+        saved = ops.forward_save(w, t, r, *s, tile=ops.TileConfig(save_counting=True, **tile))[0]
+        np.testing.assert_array_equal(P.cpu().numpy(), saved.cpu().numpy())
+        E, _ = ops.field(w, t, r, *s, 0.3, 4.0, tile=ops.TileConfig(**tile))
+        Es, _, _ = ops.field_save(w, t, r, *s, 0.3, 4.0, tile=ops.TileConfig(save_counting=True, **tile))
+        np.testing.assert_array_equal(E.cpu().numpy(), Es.cpu().numpy())
+    assert_power_close(P.cpu().numpy(), oracle_mod.power(walls, tx, rx, *s))
