@@ -113,7 +113,10 @@ __device__ __forceinline__ void sigmoid_vis_sweep(const VSmem& s, int W, const C
     }
   };
   for (int w0 = 0; w0 < W; w0 += 8) {
-    if (K == 0 && w0 + 8 <= W) {   // see WALL_TURN
+    // whole blocks of 8 walls: its kernels have no other stage to share the instruction cache
+    // with (K = 2, GB300, one wall a turn -> 8: transmitter adjoint of 64 walls x 4096
+    // receivers, alpha 100, 7.58 -> 7.23 ms; field's, alpha 10, 15.1 -> 14.8)
+    if (w0 + 8 <= W) {
 #pragma unroll
       for (int i = 0; i < 8; ++i) wall(w0 + i);
     } else {
