@@ -87,12 +87,24 @@ typedef struct {
   int32_t flags;           /* DRT_TILE_* bits */
 } drt_tile;
 
-/* Accepted for compatibility.  The forward, the coherent field and the 2D batched
-   descent leave out the obstruction loop of every path whose validity is exactly 0
-   (hard sigmoid and step outside the saturation margin: the powers are the same, bit
-   for bit) without being asked, and of the sigmoid's paths that are below 2^-26 / N_K
-   of their receiver's line of sight (N_K candidates; refl_coef >= 0): all of them
-   together are below a quarter rounding of the receiver's power. */
+/* Paths that every call leaves out, 2D and 3D, without a flag and with none against it:
+   - Hard sigmoid and unit step: paths whose validity, or some leg's visibility, is
+     exactly 0 (a saturated smoothing).  Their power and gradient are exactly 0: the
+     results are the same, bit for bit.
+   - Sigmoid with refl_coef >= 0 and max_order >= 1: paths that are negligible beside
+     their receiver's line of sight (none where that has power 0).  With N_K candidates,
+       drt_forward, drt_forward_save, drt_objective_host, drt3_forward and the batch's
+       forward: power below 2^-26 / N_K of the line of sight's (drt_field: amplitude, of
+       its amplitude), all of them together below a quarter FP32 rounding of the
+       receiver's sum;
+       drt_vjp, drt_vjp_saved, drt_field_vjp, drt_field_vjp_saved, drt3_vjp and
+       drt3_vjp_tx: 2^-50 / N_K.  A wall that only such paths touch has a gradient of
+       exactly 0 where the formula's is below 2^-50 of the others' scale.
+     drt_min_loss_vjp, the batch's adjoint and the path finders leave out exact zeros
+     alone. */
+
+/* Accepted for compatibility, without effect: paths of validity exactly 0 are left out
+   by every call (above). */
 #define DRT_TILE_CULL_INVALID 1
 
 /* Hard sigmoid and sigmoid with alpha <= 1e4: the forward holds two receivers

@@ -4,25 +4,25 @@
 //
 // Each (receiver, candidate) recomputes its image chain, reflection points, legs
 // and validity, then runs two sweeps over the walls.  Sweep 1 rebuilds each
-// leg's visibility as a product of non-zero factors plus a count of exact zeros,
-// so that the derivative of the product w.r.t. one factor never divides by zero
-// (for the sigmoid the forward can keep these visibilities instead, and the
-// SAVED variants read them in place of sweep 1).  Sweep 2 recomputes each
-// factor and pushes its adjoint into the vertices, the leg normals and the
-// wall.  The vertex and leg adjoints then flow back through the leg lengths,
+// leg's visibility; a path with a factor of exactly 0 has no gradient and stops
+// there, so sweep 2 never divides by zero (for the sigmoid the forward can keep the
+// visibilities instead, and the SAVED variants read them in place of sweep 1).  Sweep
+// 2 recomputes each factor and pushes its adjoint into the vertices, the leg normals
+// and the wall.  The vertex and leg adjoints then flow back through the leg lengths,
 // the validity, the backtrace and the image chain to the transmitter.
 //
-// The mapping is the forward's: 32 receivers per warp, one warp-uniform
-// candidate at a time; warps take their units from a counter (work stealing)
-// and store each unit's TX adjoint.  Per-wall adjoints are summed over the warp
-// with shuffles (only when a lane has a non-zero one), added into a per-CTA
-// shared-memory table, and written per CTA; a last kernel adds the CTA tables
-// in a fixed order, adds the units' TX adjoints in a fixed order, and chains the
-// per-wall quantities (n, c, t0, len) back to the end points.  The hard sigmoid and
-// the step go through drt_vjp_walk.cuh, which regroups the paths that have a gradient; the
-// sigmoid without the wall gradient, or with one receiver a lane, leaves out the paths
-// below FLOOR_VJP of the forward's floors where a whole warp's are (128 walls x 4096
-// receivers, GB300: transmitter only 99 -> 56 ms, one receiver a lane 94 -> 47).
+// A unit is a tile of receivers x a chunk of candidates; warps take their units from
+// a counter (work stealing) and store each unit's TX adjoint.  The hard sigmoid, the
+// step and the sigmoid with the wall gradient (drt_adjoint_pair.cu) go through
+// drt_vjp_walk.cuh, which queues the paths that have a gradient: their lanes hold
+// queued paths.  In the sigmoid's other forms (without the wall gradient, or one
+// receiver a lane) the lanes hold 32 receivers of one candidate at a time, and paths
+// below FLOOR_VJP of the forward's floors are left out where a whole warp's are (128
+// walls x 4096 receivers, GB300: transmitter only 99 -> 56 ms, one receiver a lane 94 ->
+// 47).  Per-wall adjoints are summed over the warp with shuffles (only when a lane has a
+// non-zero one), added into a per-CTA shared-memory table, and written per CTA; a last
+// kernel adds the CTA tables in a fixed order, adds the units' TX adjoints in a fixed
+// order, and chains the per-wall quantities (n, c, t0, len) back to the end points.
 #include <cuda_runtime.h>
 
 #include "drt_common.cuh"

@@ -14,7 +14,7 @@
 //   2. batch_argmin_kernel: loss = -min_r P_r and its argmin per problem.
 //   3. batch_adjoint_kernel: d loss / d tx for the argmin receiver of every
 //      problem; a unit is (problem, a block of warps x 32 candidates), lanes
-//      hold candidates (as in the one-receiver adjoint).
+//      hold candidates, each walking all walls.
 //   4. batch_adam_kernel: Adam on the TX position, clamped to a box.
 //   5. batch_step_end_kernel: advances the device-side step counter, which
 //      also selects the step's alpha from a schedule.

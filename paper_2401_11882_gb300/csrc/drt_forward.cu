@@ -16,7 +16,7 @@
 // receivers, 4097 sequences, hard sigmoid, alpha = 100, GB300): 20.9 ms with every path
 // evaluated, 0.8 ms with the walk; powers the same bit for bit.  The sigmoid on 64
 // walls x 32761 receivers: 22.5 ms with every path, 19.0 without the ones that underflow
-// to 0, 6.6 without the ones below the receivers' floors.
+// to 0, 6.1 without the ones below the receivers' floors.
 //
 // Hot loop (obstruction, Sec. V-A with the comparison rule x0 > x1 -> s(x0 - x1)):
 // for every wall, the smoothed side of each path vertex is computed once and

@@ -6,7 +6,7 @@
 // and selects stay per path.  The per-wall adjoints of the two paths are added in the
 // lane before the warp reduction, which is then shared by 64 paths.
 //
-// Sweep 1 is sigmoid_vis_sweep's product form without the zero count: a factor
+// Sweep 1 is sigmoid_vis_sweep's product form: a factor
 // that is exactly 0 (an FP32 underflow of the sigmoid) or a product that
 // underflows makes the leg's visibility 0, and such a path has an exactly-zero
 // gradient either way (see path_vjp), so the lane only needs to know that it is
