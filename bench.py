@@ -159,7 +159,8 @@ def file_hash(path: str) -> str:
         return hashlib.sha256(f.read()).hexdigest()[:16]
 
 
-FORWARD_SOURCES = ("drt_forward.cu", "drt_path.cuh", "drt_path_pair.cuh", "drt_common.cuh")
+FORWARD_SOURCES = ("drt_forward.cu", "drt_path.cuh", "drt_path_pair.cuh", "drt_path_queue.cuh",
+                   "drt_common.cuh")
 
 
 def forward_source_hash() -> str:
